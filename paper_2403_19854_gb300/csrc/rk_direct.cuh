@@ -1173,7 +1173,9 @@ __global__ void __launch_bounds__(RTile<T, R, SMALL>::THREADS, RTile<T, R, SMALL
     // Address and predicate instructions outnumber the sums here if they are left to the
     // inner loop: copies run through pointers that step from plane to plane, a thread
     // without an item of its own repeats the last one (the same values to the same place),
-    // and 16-byte copies and single ones are two loops.
+    // and 16-byte copies and single ones are two loops.  A CG step copies every unit once:
+    // its owner forms p in place as soon as its own copies have landed, and a second copy of
+    // the unit could land after that and leave r where p belongs.
     const int tid = rtid - D::YZT;
     static_assert(HP <= kRowPad && D::TX <= kRowTile, "padded rows of flags");
     static_assert((kStages & (kStages - 1)) == 0, "stages by masking");
@@ -1225,6 +1227,9 @@ __global__ void __launch_bounds__(RTile<T, R, SMALL>::THREADS, RTile<T, R, SMALL
           T* to = dbuf + (k & (kStages - 1)) * D::ND;
 #pragma unroll
           for (int i = 0; i < D::NLD; ++i) {
+            if constexpr (CG) {
+              if (D::XT * (i + 1) > UNITS && tid + i * D::XT >= UNITS) continue;
+            }
             if constexpr (VEC) {
               cp_async16(to + unit[i] * VL, src[i], 16);
               if constexpr (CG) cp_async16(to + kStages * D::ND + unit[i] * VL, src[i] + pdiff, 16);
