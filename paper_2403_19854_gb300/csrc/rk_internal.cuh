@@ -224,7 +224,8 @@ cudaError_t launch_mask(double* out, const double* a, const uint8_t* mask, long 
 // out = a - b
 cudaError_t launch_sub(double* out, const double* a, const double* b, long long n, cudaStream_t s);
 // a *= b (elementwise)
-cudaError_t launch_mul(double* a, const double* b, long long n, cudaStream_t s);
+template <typename T>
+cudaError_t launch_mul(T* a, const T* b, long long n, cudaStream_t s);
 // u8 -> double
 cudaError_t launch_u8_to_f64(double* out, const uint8_t* m, long long n, cudaStream_t s);
 // nonlinear reaction terms (kind 0: c u^3, 1: c sinh u, 2: c exp u)

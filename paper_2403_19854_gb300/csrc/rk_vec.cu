@@ -822,14 +822,18 @@ cudaError_t launch_mask(double* out, const double* a, const uint8_t* mask, long 
   return cudaGetLastError();
 }
 
-__global__ void k_mul(double* a, const double* b, long long n) {
+template <typename T>
+__global__ void k_mul(T* a, const T* b, long long n) {
   RK_GRID_LOOP(i, n) a[i] *= b[i];
 }
-cudaError_t launch_mul(double* a, const double* b, long long n, cudaStream_t s) {
+template <typename T>
+cudaError_t launch_mul(T* a, const T* b, long long n, cudaStream_t s) {
   count_launch();
-  k_mul<<<ew_grid(n), 256, 0, s>>>(a, b, n);
+  k_mul<T><<<ew_grid(n), 256, 0, s>>>(a, b, n);
   return cudaGetLastError();
 }
+template cudaError_t launch_mul<double>(double*, const double*, long long, cudaStream_t);
+template cudaError_t launch_mul<float>(float*, const float*, long long, cudaStream_t);
 
 __global__ void k_u8_to_f64(double* o, const uint8_t* m, long long n) {
   RK_GRID_LOOP(i, n) o[i] = m[i] ? 1.0 : 0.0;
