@@ -144,12 +144,13 @@ __global__ void __launch_bounds__(kBlockThreads) k_cell_sums(const __grid_consta
   for (int e = threadIdx.x; e < nd; e += kBlockThreads) {
     const int t = box_div(e, rwx), x = e - t * wx, z = box_div(t, rwy), y = t - z * wy;
     const long long i = ox[x] + oy[y] + oz[z];
-    T v = __ldg(a.in + i);
+    T v;
     if constexpr (CG) {
-      v += beta * p_old[i];
+      v = a.in[i] + beta * p_old[i];  // (not __ldg: the update that writes r may overlap this kernel)
       if ((unsigned)(x - R) < (unsigned)nx && (unsigned)(y - R) < (unsigned)ny && (unsigned)(z - R) < (unsigned)nz) p_new[i] = v;
-    } else if (a.in_bits) {
-      if (!(__ldg(a.flags + i) & a.in_bits)) v = (T)0;
+    } else {
+      v = __ldg(a.in + i);
+      if (a.in_bits && !(__ldg(a.flags + i) & a.in_bits)) v = (T)0;
     }
     d[e] = v;
   }

@@ -632,12 +632,10 @@ struct VecN {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(kRedThreads) k_cg_xr_fused(T* __restrict__ x, T* __restrict__ r,
-                                                            const T* p, const T* p1, const T* __restrict__ Ap,
-                                                            CGState* st, long long n, double* __restrict__ part,
-                                                            unsigned* counter) {
+__global__ void __launch_bounds__(kRedThreads) k_cg_xr_fused(T* x, T* r, const T* p, const T* p1, const T* Ap,
+                                                            CGState* st, long long n, double* part, unsigned* counter) {
   using V = VecN<T>;
-  // r, Ap and x of the thread's first vectors are on their way before alpha and p are known
+  // (no __restrict__: the operator that writes Ap may overlap this kernel, grid_wait)
   constexpr int U = 2;
   const long long nv = n / V::N, stride = (long long)gridDim.x * kRedThreads;
   grid_wait();
