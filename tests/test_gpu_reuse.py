@@ -1,0 +1,44 @@
+"""Handles used again with other options: the captured chunk of CG iterations of a batched
+solve belongs to the steps it was captured with.  The same kernels in the same order as on new
+handles, hence the same bits.
+"""
+import numpy as np
+import pytest
+
+from paper_2403_19854_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("no CUDA device", allow_module_level=True)
+
+from paper_2403_19854_gb300 import rk  # noqa: E402
+
+DEV = torch.device("cuda:0")
+
+
+def batch(p, sources):
+    H = rk.Handle.from_problem(p, device=DEV)
+    hs = [H] + [H.clone() for _ in sources[1:]]
+    new = lambda: torch.empty(p.nbox, dtype=torch.float64, device=DEV)  # noqa: E731
+    t = lambda v: torch.as_tensor(v, device=DEV)  # noqa: E731
+    return [(h, t(r), t(p.g), new(), new()) for h, r in zip(hs, sources)]
+
+
+def solve(items, precond):
+    infos = rk.solve_batched(items, precision="mixed", tol=1e-10, precond=precond)
+    return [(i["status"], i["iterations"], it[3].cpu().numpy(), it[4].cpu().numpy()) for i, it in zip(infos, items)]
+
+
+@pytest.mark.parametrize("order", [("none", "spectral", "none"), ("spectral", "none", "spectral")], ids="-".join)
+def test_batched_again_with_another_preconditioner(order):
+    p = W.cube_problem(48, 2.0, 1, "sin")
+    p.g = np.where(p.chi_gamma > 0, 0.1, 0.0)
+    sources = [p.r, np.where(p.chi > 0, W.random_field(p.nbox, 5), 0.0)]
+    fresh = {k: solve(batch(p, sources), k) for k in set(order)}
+    items = batch(p, sources)
+    for precond in order:
+        for got, ref in zip(solve(items, precond), fresh[precond]):
+            assert got[:2] == ref[:2]
+            assert np.array_equal(got[2], ref[2]) and np.array_equal(got[3], ref[3])
