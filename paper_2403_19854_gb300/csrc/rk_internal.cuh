@@ -237,7 +237,7 @@ cudaError_t launch_grad_g(double* const* g, const double* b, const double* chiV,
 // out2 = {sum_chi V w N(u + alpha w), sum_chi V w^2 N'(u + alpha w)}; partials2 holds 2 x kRedBlocks
 cudaError_t launch_nl_line(const double* u, const double* w, const double* V, const uint8_t* chi, int kind, double c,
                            double alpha, long long n, double* partials2, double* out2, cudaStream_t s);
-// y = a x + b y
+// y = a x + b y (b = 0: y is only written)
 cudaError_t launch_axpby(double* y, double a, const double* x, double b, long long n, cudaStream_t s);
 // d += dt (f - Kd) / ml where mask (forward Euler with lumped mass)
 cudaError_t launch_explicit_step(double* d, const double* f, const double* Kd, const double* ml, const uint8_t* mask,

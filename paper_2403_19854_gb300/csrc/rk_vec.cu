@@ -779,9 +779,9 @@ cudaError_t launch_add(double* d, const double* a, const double* b, long long n,
   return cudaGetLastError();
 }
 
-// y = a x + b y
+// y = a x + b y; b = 0: y is not read (it may hold anything)
 __global__ void k_axpby(double* y, double a, const double* x, double b, long long n) {
-  RK_GRID_LOOP(i, n) y[i] = a * x[i] + b * y[i];
+  RK_GRID_LOOP(i, n) y[i] = b == 0.0 ? a * x[i] : a * x[i] + b * y[i];
 }
 cudaError_t launch_axpby(double* y, double a, const double* x, double b, long long n, cudaStream_t s) {
   count_launch();

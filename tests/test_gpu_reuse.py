@@ -1,6 +1,6 @@
-"""Handles used again with other options: the captured chunk of CG iterations of a batched
-solve belongs to the steps it was captured with.  The same kernels in the same order as on new
-handles, hence the same bits.
+"""Handles used again: the captured chunk of CG iterations of a batched solve belongs to the
+steps it was captured with, and what an earlier call left in the work arrays is not read.  The
+same kernels in the same order as on new handles, hence the same bits.
 """
 import numpy as np
 import pytest
@@ -42,3 +42,18 @@ def test_batched_again_with_another_preconditioner(order):
         for got, ref in zip(solve(items, precond), fresh[precond]):
             assert got[:2] == ref[:2]
             assert np.array_equal(got[2], ref[2]) and np.array_equal(got[3], ref[3])
+
+
+def test_nonlinear_solve_after_a_failed_call():
+    """The first search direction is written over whatever the work array holds (NaN here)."""
+    p = W.cube_problem(16, 2.5, 1, "sin")
+    p.g = np.where(p.chi_gamma > 0, 0.2 * W.random_field(p.nbox, 4), 0.0)
+    r, g = torch.as_tensor(p.r, device=DEV), torch.as_tensor(p.g, device=DEV)
+    H = rk.Handle.from_problem(p, device=DEV)
+    ref = H.solve_nonlinear(r, g, "cubic", 5.0, tol=1e-8, max_iter=20000)[0]
+    H.close()
+    H = rk.Handle.from_problem(p, device=DEV)
+    with pytest.raises(rk.RKError):
+        H.transient_implicit(torch.full_like(r, float("nan")), g, 1e-3, 1, r.clone())
+    got = H.solve_nonlinear(r, g, "cubic", 5.0, tol=1e-8, max_iter=20000)[0]
+    assert torch.equal(got, ref)
