@@ -57,3 +57,19 @@ def test_nonlinear_solve_after_a_failed_call():
         H.transient_implicit(torch.full_like(r, float("nan")), g, 1e-3, 1, r.clone())
     got = H.solve_nonlinear(r, g, "cubic", 5.0, tol=1e-8, max_iter=20000)[0]
     assert torch.equal(got, ref)
+
+
+def test_clone_does_not_wait_for_the_default_stream():
+    """Work that the caller has in flight on the legacy default stream goes on."""
+    p = W.cube_problem(32, 2.0, 1, "sin")
+    H = rk.Handle.from_problem(p, device=DEV)
+    H.clone().close()
+    torch.cuda.synchronize()
+    done = torch.cuda.Event()
+    torch.cuda._sleep(int(2e9))  # about a second
+    done.record()
+    c = H.clone()
+    assert not done.query()
+    torch.cuda.synchronize()
+    d = torch.as_tensor(W.random_field(p.nbox, 3), device=DEV)
+    assert torch.equal(c.apply_K(d), H.apply_K(d))
