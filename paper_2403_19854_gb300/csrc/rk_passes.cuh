@@ -71,7 +71,7 @@ struct PassArgs {
   const cpx<T>* tw;           // twiddles of this axis, [N]
   int reflect;
   int coef_rows;              // rows of coef (2 degree + 1); 0: not staged in shared memory
-  const uint8_t* in_mask;     // optional: inputs multiplied by mask (x pass only)
+  const uint8_t* in_mask;     // optional: inputs off the mask count as zero (x pass only)
   const uint8_t* out_mask;    // optional: outputs multiplied by mask (x pass only)
   int nx, ny, nz;
   long long line_stride;      // strided passes: element stride along the line
@@ -465,6 +465,8 @@ RK_DEV T mask_of(const uint8_t* m, long long i) {
   return m ? (T)RK_LDG(m + i) : (T)1;
 }
 
+RK_DEV bool in_mask_at(const uint8_t* m, long long i) { return !m || RK_LDG(m + i) != 0; }
+
 // The mask bytes of a block's 2*LX rows form one contiguous range (rows of
 // consecutive pairs are consecutive); copy it to shared memory with 16-byte loads
 // so the threads read their bytes from there.  Requires nx % 8 == 0 (the range
@@ -694,7 +696,8 @@ __global__ void __launch_bounds__(XPass<T, N, LX>::THREADS, XPass<T, N, LX>::MIN
         const int xp = F::nat_pos(t, r);
         const T x0 = ok ? (bulk ? ra[xp] : RK_LDG(in + r0 + xp)) : (T)0;
         const T x1 = ok1 ? (bulk ? rb[xp] : RK_LDG(in + r1 + xp)) : (T)0;
-        v[r] = cmk(x0 * (T)msk[(2 * l) * N + xp], ok1 ? x1 * (T)msk[(2 * l + 1) * N + xp] : (T)0);
+        // (selected, not multiplied: what lies off the mask may be anything)
+        v[r] = cmk(msk[(2 * l) * N + xp] ? x0 : (T)0, ok1 && msk[(2 * l + 1) * N + xp] ? x1 : (T)0);
       }
     } else {
 #pragma unroll
@@ -702,8 +705,7 @@ __global__ void __launch_bounds__(XPass<T, N, LX>::THREADS, XPass<T, N, LX>::MIN
         const int xp = F::nat_pos(t, r);
         const T x0 = ok ? (bulk ? ra[xp] : RK_LDG(in + r0 + xp)) : (T)0;
         const T x1 = ok1 ? (bulk ? rb[xp] : RK_LDG(in + r1 + xp)) : (T)0;
-        v[r] = ok ? cmk(x0 * mask_of<T>(a.in_mask, r0 + xp), ok1 ? x1 * mask_of<T>(a.in_mask, r1 + xp) : (T)0)
-                  : cmk((T)0, (T)0);
+        v[r] = cmk(ok && in_mask_at(a.in_mask, r0 + xp) ? x0 : (T)0, ok1 && in_mask_at(a.in_mask, r1 + xp) ? x1 : (T)0);
       }
     }
     F::forward(v, t, buf, a.tw);
@@ -850,7 +852,7 @@ __global__ void __launch_bounds__(XPass<T, N, LX>::THREADS, XPass<T, N, LX>::MIN
 #pragma unroll
       for (int r = 0; r < X::R; ++r) {
         const int xp = F::nat_pos(t, r);
-        acc[r] = pmul(acc[r], cmk((T)msk[(2 * l) * N + xp], (T)msk[(2 * l + 1) * N + xp]));
+        acc[r] = cmk(msk[(2 * l) * N + xp] ? acc[r].x : (T)0, msk[(2 * l + 1) * N + xp] ? acc[r].y : (T)0);
       }
     if (ok)
 #pragma unroll
@@ -1110,7 +1112,7 @@ __global__ void __launch_bounds__(ZPass<T, N, L, MODE>::THREADS) k_z_fused(const
         cpx<T> wv = S::load(a.wfield, off);
         yv = pmul(yv, wv);
       }
-      if (ok && a.mask) yv = cmk(yv.x * (T)a.mask[off], yv.y * (T)a.mask[off + 1]);
+      if (ok && a.mask) yv = cmk(a.mask[off] ? yv.x : (T)0, a.mask[off + 1] ? yv.y : (T)0);
       y[r] = yv;
     }
   }
