@@ -272,22 +272,40 @@ def run_cg(args):
 #   y_split       2 in, 3 out
 #   z_merge       the z axis of Alg. 2 as its regular part: the 3 y outputs in, the 3
 #                 z outputs out (one spectral multiplier per group)
+#   stiff_pointwise  by passes the local corrections of the non-regular nodes along z (reads
+#                 and updates the fields on the boundary layers only: no per-box-node figure)
 #   y_merge       3 in, 2 out
 #   x_merge       2 in + output mask, Ap out, p in (p.Ap fused)
 #   cg_vector     x, r, p, Ap in; x, r out
-# Supports of at most four nodes to a side take K.u by direct sums, all of it in the class
-# of the pointwise stage: a CG step reads r and the last p, writes p and Ap, and reads a
-# flag byte per node.
-def pass_bytes(cls, w, s=4):
-    return {"stiff_pointwise": 4 * w + 1, "x_split": 5 * w, "y_split": 5 * w, "z_merge": 6 * w, "y_merge": 5 * w, "x_merge": 4 * w + 1,
-            "cg_vector": 6 * w}.get(cls)
+# A CG step that goes by direct sums has all of its K.u in stiff_pointwise: it reads r and the
+# last p, writes p and Ap, and reads a flag byte per node.
+def pass_bytes(cls, w, by_passes):
+    return {"stiff_pointwise": None if by_passes else 4 * w + 1, "x_split": 5 * w, "y_split": 5 * w, "z_merge": 6 * w,
+            "y_merge": 5 * w, "x_merge": 4 * w + 1, "cg_vector": 6 * w}.get(cls)
 
 
-# DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) by (class,
-# precision, size), with the sha256 of the source regions they were captured on: a
-# value holds only while those are unchanged, the traffic is null otherwise.  None has
-# been captured for K.u by direct sums.
-MEASURED_TRAFFIC = {}
+# DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the
+# kernel that dominates a step, from one ncu capture of the 256^3-box cube K.u
+# (profiles/dram_zpass_f32_cube256.md; one-pass metrics on the full-size box).
+# A value holds only while the kernel is unchanged: the sha256 of each listed
+# source region (the kernel, its block shape and its arguments) is checked at run
+# time, and the traffic is null otherwise.
+_PASSES = "paper_2403_19854_gb300/csrc/rk_passes.cuh"
+_STRIDED = (_PASSES, "template <typename T, int N, int L>\nstruct Strided {", "// PW > 0 (z SPLIT",
+            "650985d9545296426b74b48de165243a553705407e8d1c7b69a28f53a204202a")
+_SPLIT_START = ("template <typename T, int N, int L, int PW>\n__global__ void __launch_bounds__(Strided<T, N, L>::THREADS, "
+                "Strided<T, N, L>::MIN_BLOCKS_SPLIT)")
+_MERGE_START = "template <typename T, int N, int L>\n__global__ void __launch_bounds__(Strided<T, N, L>::THREADS, "
+_API = "paper_2403_19854_gb300/csrc/rk_api.cu"
+MEASURED_TRAFFIC = {
+    # the z pass (regular part of the z axis, 3 fields in, 3 out) on the split kernel
+    ("z_merge", "f32", 256): (201385472 + 144517120, [
+        _STRIDED,
+        (_PASSES, _SPLIT_START, _MERGE_START, "c68852f1a89adb44417aa6fbff51d6c92e9eccbfd5e40db56c6d0249da4d1bd0"),
+        (_API, "    // Every group has one multiplier at most, so the pass is split-shaped",
+         "    {\n      ProfScope ps(h, prof_cls<T>(RK_PROF_Z_STIFF), s);", "5c91b609926d6257cd4e52038f29fe4397c12bac9b788d54a8a258d4571fdd21"),
+    ]),
+}
 
 
 def measured_traffic(cls, prec, size):
@@ -417,7 +435,7 @@ def run_ours(args):
     (dname, dprec), (dms, dn) = dom
     w = 8 if dprec == "f64" else 4
     peak, peak_kind = _peaks()
-    bpn = pass_bytes(dname, w)
+    bpn = pass_bytes(dname, w, ("x_split", dprec) in agg)
     roofline = None
     if bpn is not None:
         traffic = args.traffic_bytes if args.traffic_bytes > 0 else measured_traffic(dname, dprec, args.size)

@@ -140,6 +140,14 @@ int rk_supported_length(int n);
  *   a_tilde    support in units of h (Eq. 64), 0.5 < a_tilde < 16
  *   stream     cudaStream_t for the set-up work (synchronised before return)
  *   out        receives the handle
+ * Operators of supports of at most four nodes to a side (a_tilde <= 5) run as direct sums or as
+ * transform passes, whichever is faster for the box, the basis, the precision and the operator;
+ * the same call on the same box always takes the same way.  What the set-up does not need is made
+ * by its first user and kept until rk_destroy: the tables and workspaces of the transform passes
+ * (the first K, solve, f^r or gradient-type force that goes by them), the preconditioner's tables
+ * (the first preconditioned solve or rk_apply_precond), the solvers' vectors.  Where a box could do
+ * without the passes, a first call that finds no memory for them, or that is being captured into
+ * a CUDA graph, runs by direct sums.
  * Errors: RK_ERR_INVALID_ARG, RK_ERR_UNSUPPORTED (size not built, odd sizes, gap
  * narrower than Eq. 66, a 1D side not a multiple of 4), RK_ERR_OOM, RK_ERR_CUDA, RK_ERR_SINGULAR_MOMENT (the
  * handle is still returned; rk_singular_nodes gives the count and first node).

@@ -104,11 +104,16 @@ constexpr RK_HD bool even_p(int p) {
   return S == 10 ? (p == 0 || p == 4 || p == 7 || p == 9) : (S == 6 ? (p == 0 || p == 3 || p == 5) : p == 0);
 }
 
-// What a launch would do: the partials p . Ap it writes, and whether K takes the way through
-// the fields g_p (on entry: whether the handle has or could have them).
+// What a launch would do: the partials p . Ap it writes, whether K takes the way through the
+// fields g_p (on entry: whether the handle has or could have them), and the time it takes on a
+// box with that share of its cells active (not empty of chi nodes; 0: not estimated, a way
+// that the transform passes do not beat).
 struct DirectQuery {
   long long blocks = 0;
   bool fields = false;
+  bool cg = true;
+  double active = 1.0;
+  double us = 0.0;
 };
 
 template <typename T>

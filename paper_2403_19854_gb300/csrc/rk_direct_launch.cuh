@@ -4,6 +4,7 @@
 #pragma once
 
 #include <algorithm>
+#include <cmath>
 
 #include "rk_cells.cuh"
 #include "rk_direct.cuh"
@@ -19,6 +20,8 @@ struct DirectPlan {
   int zc, tiles_x, tiles_y;
   long long blocks;
   double cost;
+  int steps, occ;   // steps of a block, blocks that an SM holds
+  double lat, col;  // cycles of a step: its latency, its issue time
 };
 
 // Cost of a launch in SM cycles: every block walks its planes plus those of its halo, an SM
@@ -29,7 +32,7 @@ struct DirectPlan {
 template <int TX, int TY>
 inline DirectPlan walk_plan(bool small_tile, int nx, int ny, int nz, int zmin, int halo, int occ, double lat, double col,
                             bool twos = false) {
-  DirectPlan best{small_tile, 0, (nx + TX - 1) / TX, (ny + TY - 1) / TY, 0, 0.0};
+  DirectPlan best{small_tile, 0, (nx + TX - 1) / TX, (ny + TY - 1) / TY, 0, 0.0, 0, occ, lat, col};
   const long long tiles = (long long)best.tiles_x * best.tiles_y;
   for (int zc = zmin; zc <= 256; zc += twos || zc < kCell ? zc : kCell) {
     const int c = std::min(zc, nz);
@@ -42,10 +45,40 @@ inline DirectPlan walk_plan(bool small_tile, int nx, int ny, int nz, int zmin, i
       best.zc = c;
       best.blocks = blocks;
       best.cost = t;
+      best.steps = steps;
     }
     if (c == nz) break;
   }
   return best;
+}
+
+// Times in microseconds, for the choice between direct sums and transform passes.  The costs
+// above order the ways to the direct sums; these are fits to measured calls (boxes of 36^3 to
+// 256^3, cubic and not, a cube or spheres in them; 10 % off at most places): the walk of a plan
+// with its empty cells left out (their blocks end at once; the others hold some of them), times
+// and plus what the fits give per kernel.  K with r <= 2 in FP64, r <= 3 in FP32 and every u^h
+// were faster than the passes on all of these boxes (0.2 to 0.95 times) and are not estimated.
+inline double walk_us(const DirectPlan& p, double active) {
+  const double per_sm = (double)((p.blocks + kSMs - 1) / kSMs) * std::sqrt(active);
+  return std::max(std::max(1.0, per_sm / p.occ) * p.steps * p.lat, per_sm * p.steps * p.col) / 2000.0;
+}
+// a CG step in FP32 by k_direct
+template <int S, int R>
+double direct_cg_us(const DirectPlan& p, double active) {
+  const double k = R <= 2 ? (S == 4 ? 1.35 : 1.1) : (R == 3 ? 2.0 : (S == 4 ? 1.16 : 2.25));
+  return (R <= 2 ? 5.0 : 0.0) + k * walk_us(p, active);
+}
+template <typename T, int S, int R>
+double regular_us(const DirectPlan& q, double active, int ncells, int ocells) {
+  // (in FP64 few cells leave as many long blocks: the 0.3rd power of their share)
+  const double cells = (ncells + ocells) / (2.0 * kSMs), w = walk_us(q, sizeof(T) == 8 ? std::pow(active, 0.6) : active);
+  if constexpr (sizeof(T) == 8) {
+    if (R == 3) return S == 4 ? 154.0 + 1.45 * w + 11.6 * cells : 115.0 + w + 67.0 * cells;
+    if (R == 4) return S == 4 ? 94.0 + 0.89 * w + 76.0 * cells : 85.0 + 0.82 * w + 131.0 * cells;
+  } else if (R == 4) {
+    return S == 4 ? 20.0 + 11.5 * cells : 22.0 + 0.44 * w + 14.2 * cells;
+  }
+  return 0.0;
 }
 
 // The regular stencil: cycles per step of a tile (its columns) and its latency.  Measured at
@@ -167,6 +200,19 @@ CellPlan cell_plan(int nx, int ny, int nz) {
   return best;
 }
 
+template <typename T, int S, int R, int MODE>
+double cells_us(const CellPlan& c, double active) {
+  constexpr bool F64 = sizeof(T) == 8;
+  const double t = c.cost / 2000.0;
+  if constexpr (MODE == DM_TRANSPOSE_U) {
+    if (!F64 || R < 3 || (R == 3 && S == 4)) return 0.0;
+    const double w = t * std::pow(active, 0.7);
+    return R == 3 ? 52.0 + 0.67 * w : (S == 4 ? 25.0 + 0.94 * w : 70.0 + 0.72 * w);
+  }
+  if constexpr (MODE == DM_STIFF) return F64 ? (R >= 3 ? 20.0 + 1.02 * t * std::pow(active, 0.7) : 0.0) : (R >= 2 ? 8.0 + 0.72 * t * std::sqrt(active) : 0.0);
+  return 0.0;
+}
+
 template <typename T, int S, int R, int MODE, bool CG>
 cudaError_t cell_launch(const DirectArgs<T>& a0, const CellPlan& p, cudaStream_t s) {
   DirectArgs<T> a = a0;
@@ -222,6 +268,8 @@ cudaError_t direct_mode(const DirectArgs<T>& a0, cudaStream_t s, DirectQuery* qu
       // smallest eigenvalues lie near the rounding (a = 2.5: T_0 nearly vanishes at the highest
       // frequencies) CG needs more steps.  a = 2.5, 256^3 cube, mixed solve to 1e-10: 1625
       // iterations, 1.31 s, against 6675, 2.5 s (128^3 2250 / 2950); r = 1: as many both ways.
+      // On such large boxes the transform passes are faster still (1825 iterations, 1.00 s;
+      // choose_routes weighs them).
       constexpr bool product = CG && sizeof(T) == 4 && R >= 2;
       const bool regular = !product && a.corrected && q.cost + ccost < direct;
       cells = (query ? query->fields : a.gall != nullptr) && c.cost < (regular ? q.cost + ccost : direct);
@@ -230,6 +278,7 @@ cudaError_t direct_mode(const DirectArgs<T>& a0, cudaStream_t s, DirectQuery* qu
         if (query) {
           query->fields = false;
           query->blocks = a.parts;
+          query->us = regular_us<T, S, R>(q, query->active, corr ? a.ncells : 0, corr ? a.ocells : 0);
           return cudaSuccess;
         }
         cudaError_t e = q.small_tile ? regular_launch<T, R, true, CG>(a, q, s) : regular_launch<T, R, false, CG>(a, q, s);
@@ -243,6 +292,7 @@ cudaError_t direct_mode(const DirectArgs<T>& a0, cudaStream_t s, DirectQuery* qu
       if (query) {
         query->fields = true;
         query->blocks = a.parts;
+        query->us = cells_us<T, S, R, MODE>(c, query->active);
         return cudaSuccess;
       }
       return cell_launch<T, S, R, MODE, CG>(a, c, s);
@@ -254,6 +304,7 @@ cudaError_t direct_mode(const DirectArgs<T>& a0, cudaStream_t s, DirectQuery* qu
     if (query) {
       query->fields = false;
       query->blocks = p.blocks;
+      query->us = CG && sizeof(T) == 4 && R >= 2 ? direct_cg_us<S, R>(p, query->active) : 0.0;
       return cudaSuccess;
     }
     if constexpr (DBasis<S>::DIM == 3) {
@@ -267,7 +318,7 @@ cudaError_t direct_mode(const DirectArgs<T>& a0, cudaStream_t s, DirectQuery* qu
 template <typename T, int S, int R>
 cudaError_t direct_s(int mode, const DirectArgs<T>& a, cudaStream_t s, DirectQuery* query) {
   switch (mode) {
-    case DM_STIFF: return a.cg || query ? direct_mode<T, S, R, DM_STIFF, true>(a, s, query) : direct_mode<T, S, R, DM_STIFF, false>(a, s, query);
+    case DM_STIFF: return a.cg || (query && query->cg) ? direct_mode<T, S, R, DM_STIFF, true>(a, s, query) : direct_mode<T, S, R, DM_STIFF, false>(a, s, query);
     case DM_MASS_STIFF:
       if constexpr (DBasis<S>::DIM == 3 && sizeof(T) == 8) {
         if (!a.gall || !a.cg || query) return cudaErrorInvalidValue;
