@@ -63,7 +63,7 @@ typedef enum rk_dtype { RK_F64 = 0, RK_F32 = 1 } rk_dtype;
 
 typedef enum rk_precision {
   RK_PREC_FP64 = 0,  /* every convolution and CG vector in FP64 */
-  RK_PREC_MIXED = 1  /* FP32 convolutions and CG vectors, FP64 dots, FP64 refinement */
+  RK_PREC_MIXED = 1  /* FP32 convolutions and CG vectors, dot products to FP64 accuracy, FP64 refinement */
 } rk_precision;
 
 typedef struct rk_grid {
@@ -208,7 +208,7 @@ rk_status rk_get_shape(const rk_handle* h, int32_t n[3], int32_t* s, int64_t* n_
  * conjugate gradients solve chi_Omega o K(chi_Omega o x) = F with
  * F = chi_Omega o (f^r - K d_Gamma) until ||F - A x|| <= tol ||F|| (FP64
  * residual); then u^h = Alg. 3 (d).  In RK_PREC_MIXED the CG runs in FP32
- * (FP32 convolutions and vectors, FP64 dot products) and its residual is
+ * (FP32 convolutions and vectors, dot products as accurate as FP64 sums) and its residual is
  * periodically replaced by the true FP64 residual (FP64 operator), the FP32
  * correction being accumulated into the FP64 iterate (iterative refinement
  * without restarting the Krylov recurrence).
@@ -350,15 +350,15 @@ enum {
   RK_PROF_Y_SPLIT = 1,       /* y pass, forward chain */
   RK_PROF_Z_SPLIT = 2,       /* z pass, forward chain (set-up moments; in Alg. 2 it also applies
                                 the pointwise stage to the regular nodes when n_x % 4 == 0) */
-  RK_PROF_Z_STIFF = 3,       /* K.u by direct sums (supports of at most four nodes to a side), all
-                                its kernels; else the pointwise stage of Alg. 2 (Eq. 90-91) */
+  RK_PROF_Z_STIFF = 3,       /* K.u by direct sums, all its kernels; by transform passes the pointwise
+                                stage of Alg. 2 (Eq. 90-91) or the local corrections along z */
   RK_PROF_Z_EVAL_U = 4,      /* Alg. 3 by direct sums, else its fused z pass */
   RK_PROF_Z_TRANSPOSE_U = 5, /* Alg. 4 / transpose of Alg. 3 by direct sums, else the fused z pass */
   RK_PROF_Y_MERGE = 6,       /* y pass, reflected chain */
   RK_PROF_X_MERGE = 7,       /* x pass, reflected chain */
   RK_PROF_MOMENT_SOLVE = 8,  /* per-node M^{-1} of Alg. 1 */
   RK_PROF_CG_VECTOR = 9,     /* CG dot products and vector updates (per iteration) */
-  RK_PROF_Z_MERGE = 10,      /* z pass, reflected chain */
+  RK_PROF_Z_MERGE = 10,      /* z pass, reflected chain, or the regular part of the z axis (both in one) */
   RK_PROF_PRECOND = 11,      /* spectral preconditioner (five passes) */
   RK_PROF_CLASSES = 12
 };

@@ -132,7 +132,6 @@ struct DirectArgs {
   int diag;              // b^k of a regular node is diagonal (g_{1+k} = creg[k] D_{1+k})
   T creg[3];
   const T* b0;           // b^0_p fields, [S][nbox]
-  const T* chiV;
   int diag0;             // b^0 of a regular node is zero but for the even p
   T b0reg[10];
   T vreg;                // chi V of a regular node

@@ -63,6 +63,21 @@ def test_fused_steps(box, a, deg, prec):
         p.r = np.where(p.chi > 0, np.random.default_rng(7).standard_normal(p.nbox), 0.0)
     else:
         p = problem(box, a, deg)
+    check(p, prec)
+
+
+@pytest.mark.parametrize("box,a,deg,prec", [((162, 96, 100), 1.5, 1, "mixed"), ((162, 36, 48), 2.5, 1, "mixed"),
+                                            ((48, 36, 32), 4.5, 1, "mixed"), ((64, 72, 64), 2.5, 1, "fp64"),
+                                            ((72, 100, 128), 3.0, 2, "fp64")], ids=lambda v: str(v).replace(" ", ""))
+def test_fused_steps_across_the_periodic_boundary(box, a, deg, prec):
+    p = problem(box, a, deg)
+    shift = (box[2] - 3, box[1] // 2, 5)
+    for k in ("chi", "chi_gamma", "V", "r", "g"):
+        setattr(p, k, np.roll(getattr(p, k).reshape(box[2], box[1], box[0]), shift, axis=(0, 1, 2)).reshape(-1))
+    check(p, prec)
+
+
+def check(p, prec):
     H = rk.Handle.from_problem(p, device=DEV)
     ref = cg(H, p, STEPS).cpu().numpy()
     r, g = torch.as_tensor(p.r, device=DEV), torch.as_tensor(p.g, device=DEV)
