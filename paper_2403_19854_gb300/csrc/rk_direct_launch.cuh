@@ -62,9 +62,10 @@ inline double walk_us(const DirectPlan& p, double active) {
   const double per_sm = (double)((p.blocks + kSMs - 1) / kSMs) * std::sqrt(active);
   return std::max(std::max(1.0, per_sm / p.occ) * p.steps * p.lat, per_sm * p.steps * p.col) / 2000.0;
 }
-// a CG step in FP32 by k_direct
+// a CG step in FP32 by k_direct (the longer walks of the quadratic basis gain more from empty cells)
 template <int S, int R>
-double direct_cg_us(const DirectPlan& p, double active) {
+double direct_cg_us(const DirectPlan& p, double share) {
+  const double active = S == 4 ? share : std::pow(share, 1.4);
   const double k = R <= 2 ? (S == 4 ? 1.35 : 1.1) : (R == 3 ? 2.0 : (S == 4 ? 1.16 : 2.25));
   return (R <= 2 ? 5.0 : 0.0) + k * walk_us(p, active);
 }
