@@ -56,8 +56,9 @@ inline DirectPlan walk_plan(bool small_tile, int nx, int ny, int nz, int zmin, i
 // above order the ways to the direct sums; these are fits to measured calls (boxes of 36^3 to
 // 256^3, cubic and not, a cube or spheres in them; 10 % off at most places): the walk of a plan
 // with its empty cells left out (their blocks end at once; the others hold some of them), times
-// and plus what the fits give per kernel.  K with r <= 2 in FP64, r <= 3 in FP32 and every u^h
-// were faster than the passes on all of these boxes (0.2 to 0.95 times) and are not estimated.
+// and plus what the fits give per kernel.  K with r <= 2 in FP64 and every u^h were faster than
+// the passes on all of these boxes (0.2 to 0.95 times) and are not estimated, nor is K in FP32
+// outside CG.
 inline double walk_us(const DirectPlan& p, double active) {
   const double per_sm = (double)((p.blocks + kSMs - 1) / kSMs) * std::sqrt(active);
   return std::max(std::max(1.0, per_sm / p.occ) * p.steps * p.lat, per_sm * p.steps * p.col) / 2000.0;
@@ -71,13 +72,11 @@ double direct_cg_us(const DirectPlan& p, double share) {
 }
 template <typename T, int S, int R>
 double regular_us(const DirectPlan& q, double active, int ncells, int ocells) {
-  // (in FP64 few cells leave as many long blocks: the 0.3rd power of their share)
-  const double cells = (ncells + ocells) / (2.0 * kSMs), w = walk_us(q, sizeof(T) == 8 ? std::pow(active, 0.6) : active);
   if constexpr (sizeof(T) == 8) {
+    // (few cells leave as many long blocks: the 0.3rd power of their share)
+    const double cells = (ncells + ocells) / (2.0 * kSMs), w = walk_us(q, std::pow(active, 0.6));
     if (R == 3) return S == 4 ? 154.0 + 1.45 * w + 11.6 * cells : 115.0 + w + 67.0 * cells;
     if (R == 4) return S == 4 ? 94.0 + 0.89 * w + 76.0 * cells : 85.0 + 0.82 * w + 131.0 * cells;
-  } else if (R == 4) {
-    return S == 4 ? 20.0 + 11.5 * cells : 22.0 + 0.44 * w + 14.2 * cells;
   }
   return 0.0;
 }

@@ -42,7 +42,8 @@ def steps(H, p, prec):
 ROUTES = [((256, 256, 256), 2.5, 1, (False, False, True, False)), ((128, 128, 128), 1.5, 1, (False, False, False, False)),
           ((96, 96, 96), 2.5, 1, (False, False, False, False)), ((144, 144, 144), 3.5, 1, (False, False, True, False)),
           ((64, 64, 64), 4.5, 2, (False, True, None, True)), ((128, 128, 128), 4.5, 2, (None, None, True, True)),
-          ((96, 96, 96), 4.5, 1, (None, True, None, None))]
+          ((96, 96, 96), 4.5, 1, (False, True, None, False)), ((128, 128, 128), 4.5, 1, (False, True, None, None)),
+          ((144, 144, 144), 4.5, 1, (False, None, None, False))]
 
 
 @pytest.mark.parametrize("box,a,deg,want", ROUTES, ids=lambda v: str(v).replace(" ", ""))
